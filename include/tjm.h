@@ -323,6 +323,15 @@ tjm_status tjm_selftest_qr(int double_precision, int m, int n, const double* A, 
  * the truncations of Sec. "1TDVP and 2TDVP as tensor networks". */
 tjm_status tjm_selftest_svd(int double_precision, int m, int n, const double* A, double* U, double* S, double* V);
 
+/* The same SVD as a truncation asks for it that discards up to a share cut >= 0
+ * of the squared singular values (trunc_eps): directions of at most
+ * min(cut, 1/2) / nn^2 of their sum are not told apart, so the trailing columns
+ * that the truncation discards need not be singular vectors.  Its rank, the
+ * values and columns it keeps and the sum of squares are those of cut = 0.
+ * TJM_EINVAL for a negative cut. */
+tjm_status tjm_selftest_svd_cut(int double_precision, int m, int n, double cut, const double* A, double* U, double* S,
+                                double* V);
+
 /* C = op(A) op(B) on the tensor cores (tcgen05, TF32 inputs with the 3xTF32
  * split, FP32 accumulation in tensor memory), one CTA: the complex GEMM of
  * the effective-Hamiltonian and environment contractions (Fig. 2 networks).

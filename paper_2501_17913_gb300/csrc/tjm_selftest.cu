@@ -42,10 +42,11 @@ qr_test_kernel(int m, int n, const cx<double>* A, cx<double>* Q, cx<double>* R, 
 
 template <class T>
 __global__ void __launch_bounds__(TJM_THREADS, 1)
-svd_test_kernel(int m, int n, const cx<double>* A, cx<double>* U, double* S, cx<double>* V, cx<T>* ws, int* iw) {
+svd_test_kernel(int m, int n, const cx<double>* A, cx<double>* U, double* S, cx<double>* V, cx<T>* ws, int* iw,
+                double cut) {
   __shared__ double red[TJM_WARPS * 64];
   __shared__ __align__(16) char psm[kSvdSmem];
-  svd_call_body<T>(m, n, A, U, S, V, ws, iw, red, psm);
+  svd_call_body<T>(m, n, A, U, S, V, ws, iw, red, psm, cut);
 }
 
 // C = op(A) op(B) on the tensor cores, one CTA.  A is given row-major M x K,
@@ -135,7 +136,12 @@ tjm_status tjm_selftest_qr(int double_precision, int m, int n, const double* A, 
 }
 
 tjm_status tjm_selftest_svd(int double_precision, int m, int n, const double* A, double* U, double* S, double* V) {
-  if (m < 1 || n < 1 || m > 256 || n > 256 || !A || !U || !S || !V) return TJM_EINVAL;
+  return tjm_selftest_svd_cut(double_precision, m, n, 0.0, A, U, S, V);
+}
+
+tjm_status tjm_selftest_svd_cut(int double_precision, int m, int n, double cut, const double* A, double* U, double* S,
+                                double* V) {
+  if (m < 1 || n < 1 || m > 256 || n > 256 || !(cut >= 0) || !A || !U || !S || !V) return TJM_EINVAL;
   const int mm = m > n ? m : n, nn = m < n ? m : n;
   Dev d;
   auto* dA = d.get<tjm::cx<double>>(m * n);
@@ -148,11 +154,12 @@ tjm_status tjm_selftest_svd(int double_precision, int m, int n, const double* A,
   if (cudaMemcpy(dA, A, (size_t)m * n * 16, cudaMemcpyHostToDevice) != cudaSuccess) return TJM_ECUDA;
   if (double_precision == 2)
     tjm::svd_test_kernel<tjm::df64><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV,
-                                                        reinterpret_cast<tjm::cx<tjm::df64>*>(ws), iw);
+                                                        reinterpret_cast<tjm::cx<tjm::df64>*>(ws), iw, cut);
   else if (double_precision)
-    tjm::svd_test_kernel<double><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV, reinterpret_cast<tjm::cx<double>*>(ws), iw);
+    tjm::svd_test_kernel<double><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV, reinterpret_cast<tjm::cx<double>*>(ws), iw,
+                                                 cut);
   else
-    tjm::svd_test_kernel<float><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV, reinterpret_cast<tjm::cx<float>*>(ws), iw);
+    tjm::svd_test_kernel<float><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV, reinterpret_cast<tjm::cx<float>*>(ws), iw, cut);
   if (finish()) return TJM_ECUDA;
   cudaMemcpy(U, dU, (size_t)m * nn * 16, cudaMemcpyDeviceToHost);
   cudaMemcpy(V, dV, (size_t)n * nn * 16, cudaMemcpyDeviceToHost);

@@ -108,6 +108,8 @@ SIGNATURES = [
                                   C.POINTER(C.c_double)]),
     ("tjm_selftest_svd", C.c_int, [C.c_int, C.c_int, C.c_int, C.POINTER(C.c_double), C.POINTER(C.c_double),
                                    C.POINTER(C.c_double), C.POINTER(C.c_double)]),
+    ("tjm_selftest_svd_cut", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_double, C.POINTER(C.c_double),
+                                       C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double)]),
     ("tjm_selftest_tc_cgemm", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
                                         C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double)]),
     ("tjm_selftest_contract", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
@@ -408,9 +410,10 @@ def selftest_qr(A, double_precision=True):
     return _z(Q), _z(R)
 
 
-def selftest_svd(A, double_precision=True):
+def selftest_svd(A, double_precision=True, cut=0.0):
     """SVD of one matrix by the kernel's block routine: returns (U, S, V) with A = U diag(S) V^H.
-    double_precision: False/0 FP32, True/1 FP64, 2 double-float emulated FP64."""
+    double_precision: False/0 FP32, True/1 FP64, 2 double-float emulated FP64.  cut: the share of the squared
+    singular values that a truncation of the result may discard (tjm_selftest_svd_cut)."""
     lib = load()
     A = np.asarray(A, dtype=np.complex128)
     m, n = A.shape
@@ -419,9 +422,9 @@ def selftest_svd(A, double_precision=True):
     U = np.zeros((m, nn, 2))
     V = np.zeros((n, nn, 2))
     S = np.zeros(nn)
-    st = lib.tjm_selftest_svd(int(double_precision), m, n, _dp(a), _dp(U), _dp(S), _dp(V))
+    st = lib.tjm_selftest_svd_cut(int(double_precision), m, n, float(cut), _dp(a), _dp(U), _dp(S), _dp(V))
     if st != TJM_OK:
-        raise TJMError(st, "tjm_selftest_svd")
+        raise TJMError(st, "tjm_selftest_svd_cut")
     return _z(U), S, _z(V)
 
 
