@@ -39,3 +39,34 @@ def test_factorizations_of_large_and_small_matrices(m, n, size, dp):
     assert np.abs(Q.conj().T @ Q - np.eye(k)).max() <= 10 * tol
     assert np.abs(Q @ (R / size) - A).max() <= tol * ref[0]
     assert np.abs(np.tril(R, -1)).max() == 0.0
+
+
+# largest squared norms just below the last binade of the range that holds them (dp 0 and 2: FP32, 2^127 = 1.7e38; dp 1:
+# FP64, 2^1023 = 9.0e307) and in it
+TOP = {0: [1.2e19, 1.35e19, 1.7e19], 1: [8e153, 1.0e154, 1.2e154], 2: [1.2e19, 1.35e19, 1.7e19]}
+
+
+@pytest.mark.parametrize("dp", [0, 1, 2])
+@pytest.mark.parametrize("m", [2, 20])
+def test_rotations_at_the_top_of_the_exponent_range(m, dp):
+    lib_ready()
+    rng = np.random.default_rng(m)
+    for size in TOP[dp]:
+        A = 1e-3 * _rand(rng, m, 2)
+        A[0], A[1] = [1.0, 0.1j], [0.0, 0.3]
+        ref = np.linalg.svd(A, compute_uv=False)
+        U, S, V = tjm.selftest_svd(A * size, dp)
+        assert np.abs(S / size - ref).max() <= TOL[dp] * ref[0]
+        assert np.abs((U * (S / size)) @ V.conj().T - A).max() <= TOL[dp] * ref[0]
+        assert np.abs(U.conj().T @ U - np.eye(2)).max() <= 10 * TOL[dp]
+
+
+@pytest.mark.parametrize("size", [1e-18, 1e-19])
+def test_rotations_at_the_bottom_of_the_exponent_range(size):
+    """Squared norms of 1e-36 and 1e-38 (the second below the normal range, with 20 bits left)."""
+    lib_ready()
+    A = np.array([[1.0, 0.1j], [0.0, 0.3]])
+    ref = np.linalg.svd(A, compute_uv=False)
+    U, S, V = tjm.selftest_svd(A * size, 0)
+    assert np.abs(S / size - ref).max() <= (TOL[0] if size > 5e-19 else 1e-3) * ref[0]
+    assert np.abs(V.conj().T @ V - np.eye(2)).max() <= 10 * TOL[0]
