@@ -185,7 +185,10 @@ __device__ __noinline__ void gemm_core(int batch, int M, int N, int K, const cx<
 // Small products: every thread forms whole outputs, reading its operands where
 // they are (the working set of a small bond sits in L1 and L2), so there is no
 // staging, no barrier before the last and no padding; consecutive threads own
-// consecutive j of as many rows as fit the CTA, one index division per thread.
+// consecutive j of as many rows as fit the CTA, one index division per thread; rows
+// longer than the CTA are dealt by flat index (taken one row at a time, the last pass over
+// 320 columns has 64 of the 256 threads: FP64 64 x 320 x 128 7.28 M cycles with one CTA per SM
+// instead of 5.66 M, 11.8 instead of 10.8 M with two).
 // Bound by instruction issue (an output's index arithmetic used to cost as much as
 // eight of its multiply-adds; two or four outputs of a thread along together, for
 // more loads in flight, were 10 % slower).
@@ -193,27 +196,29 @@ template <class T, bool CONJ>
 __device__ __forceinline__ void direct_rows(int batch, int M, int N, int K, const cx<T>* __restrict__ A, int sai, int sak,
                                             int ca, long long sa, const cx<T>* __restrict__ B, int sbk, int sbj, int cb,
                                             long long sb, cx<T>* C, int sci, int scj, long long sc) {
-  const int rows = N < TJM_THREADS ? TJM_THREADS / N : 1;
-  const int ti = threadIdx.x / N, tj = threadIdx.x - ti * N;
-  if (ti >= rows) return;
   const int MB = batch * M;
-  for (int ib = ti; ib < MB; ib += rows) {
+  auto one = [&](int ib, int j) {
     const int bt = batch == 1 ? 0 : ib / M, i = ib - bt * M;
-    for (int j = tj; j < N; j += TJM_THREADS) {      // more than once only for N > TJM_THREADS
-      const cx<T>* a = A + bt * sa + i * sai;
-      const cx<T>* b = B + bt * sb + j * sbj;
-      cx<T> acc = czero<T>();
+    const cx<T>* a = A + bt * sa + i * sai;
+    const cx<T>* b = B + bt * sb + j * sbj;
+    cx<T> acc = czero<T>();
 #pragma unroll 4
-      for (int k = 0; k < K; ++k) {
-        cx<T> x = *a, y = *b;
-        a += sak;
-        b += sbk;
-        if (CONJ) { x.y = flip(x.y, ca); y.y = flip(y.y, cb); }
-        cfma(acc, x, y);
-      }
-      C[bt * sc + i * sci + j * scj] = acc;
+    for (int k = 0; k < K; ++k) {
+      cx<T> x = *a, y = *b;
+      a += sak;
+      b += sbk;
+      if (CONJ) { x.y = flip(x.y, ca); y.y = flip(y.y, cb); }
+      cfma(acc, x, y);
     }
+    C[bt * sc + i * sci + j * scj] = acc;
+  };
+  if (N > TJM_THREADS) {
+    for (int e = threadIdx.x; e < MB * N; e += TJM_THREADS) one(e / N, e % N);
+    return;
   }
+  const int rows = TJM_THREADS / N, ti = threadIdx.x / N, j = threadIdx.x - ti * N;
+  if (ti >= rows) return;
+  for (int ib = ti; ib < MB; ib += rows) one(ib, j);
 }
 template <class T>
 __device__ __noinline__ void gemm_direct(int batch, int M, int N, int K, const cx<T>* __restrict__ A, int sai, int sak,
@@ -231,7 +236,12 @@ __device__ __noinline__ void gemm_direct(int batch, int M, int N, int K, const c
 // FP64 is bound by its unit, 2 multiply-adds per clock and SM, in which a lane without
 // an output costs as much as one with: the direct form has none but in its last warp
 // (40 x 16 x 8 19.7 k against 22.9 k cycles in tiles without padding and 213 k with, 80 x 32 x 16
-// 145 / 153 / 424 k, 160 x 64 x 32 1178 / 1180 / 1257 k), so every FP64 product takes it.
+// 145 / 153 / 424 k, 160 x 64 x 32 1178 / 1180 / 1257 k, means over two CTAs per SM).  At the largest
+// products both are at the unit (bond 64, two CTAs per SM, the later one: 320 x 128 x 64 10.7 M cycles against
+// 10.8 M in whole tiles, 128 x 64 x 320 10.7 / 10.7, 64 x 320 x 128 10.8 / 10.7; least possible 10.5), and with
+// one CTA per SM the direct form waits a little on operands that L1 does not hold (5.67 / 5.44, 5.55 / 5.44, 5.66 / 5.39;
+// least possible 5.24).  Whole FP64 runs at bond 64, one step of L = 16: 1.55 against 1.97 s with one
+// trajectory per SM, 2.77 against 3.57 with two.  So every FP64 product takes it.
 constexpr long long kDirectF32 = 8192, kOnePassF32 = 16384;
 
 // Tile choice of the tiled form.  gemm_tile_rule == 0: always 64 x 64 tiles.
