@@ -238,7 +238,8 @@ typedef struct {
   int64_t final_bond_sum;                    /* sum over trajectories and bonds of the bond dimension */
   int64_t final_bond_max;
   double flops_contract;                     /* real flops of all tensor contractions (8 per complex MAC) */
-  double flops_decomp;                       /* real flops of the QR / SVD factorizations */
+  double flops_decomp;                       /* real flops of the QR / SVD factorizations (8 per complex MAC; of the
+                                              * SVD the products formed, the rotations made and the FP32 start) */
   uint64_t cycles[12];                       /* SM cycles summed over trajectories, by phase: GEMM, MPO
                                                 contraction, Lanczos, QR, SVD, dissipation+jump, measurement,
                                                 TDVP sweep, environment build, Krylov exponential, matvec
@@ -328,9 +329,10 @@ tjm_status tjm_selftest_svd(int double_precision, int m, int n, const double* A,
  * min(cut, 1/2) / nn^2 of their sum are not told apart, so the trailing columns
  * that the truncation discards need not be singular vectors.  Its rank, the
  * values and columns it keeps and the sum of squares are those of cut = 0.
+ * flops (may be NULL) receives its real flops as tjm_stats counts them.
  * TJM_EINVAL for a negative cut. */
 tjm_status tjm_selftest_svd_cut(int double_precision, int m, int n, double cut, const double* A, double* U, double* S,
-                                double* V);
+                                double* V, double* flops);
 
 /* C = op(A) op(B) on the tensor cores (tcgen05, TF32 inputs with the 3xTF32
  * split, FP32 accumulation in tensor memory), one CTA: the complex GEMM of

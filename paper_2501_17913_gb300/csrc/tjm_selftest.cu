@@ -43,10 +43,11 @@ qr_test_kernel(int m, int n, const cx<double>* A, cx<double>* Q, cx<double>* R, 
 template <class T>
 __global__ void __launch_bounds__(TJM_THREADS, 1)
 svd_test_kernel(int m, int n, const cx<double>* A, cx<double>* U, double* S, cx<double>* V, cx<T>* ws, int* iw,
-                double cut) {
+                double cut, double* flops) {
   __shared__ double red[TJM_WARPS * 64];
   __shared__ __align__(16) char psm[kSvdSmem];
-  svd_call_body<T>(m, n, A, U, S, V, ws, iw, red, psm, cut);
+  const long long cmacs = svd_call_body<T>(m, n, A, U, S, V, ws, iw, red, psm, cut);
+  if (threadIdx.x == 0) *flops = 8.0 * (double)cmacs;
 }
 
 // C = op(A) op(B) on the tensor cores, one CTA.  A is given row-major M x K,
@@ -136,34 +137,35 @@ tjm_status tjm_selftest_qr(int double_precision, int m, int n, const double* A, 
 }
 
 tjm_status tjm_selftest_svd(int double_precision, int m, int n, const double* A, double* U, double* S, double* V) {
-  return tjm_selftest_svd_cut(double_precision, m, n, 0.0, A, U, S, V);
+  return tjm_selftest_svd_cut(double_precision, m, n, 0.0, A, U, S, V, nullptr);
 }
 
 tjm_status tjm_selftest_svd_cut(int double_precision, int m, int n, double cut, const double* A, double* U, double* S,
-                                double* V) {
+                                double* V, double* flops) {
   if (m < 1 || n < 1 || m > 256 || n > 256 || !(cut >= 0) || !A || !U || !S || !V) return TJM_EINVAL;
   const int mm = m > n ? m : n, nn = m < n ? m : n;
   Dev d;
   auto* dA = d.get<tjm::cx<double>>(m * n);
   auto* dU = d.get<tjm::cx<double>>(m * nn);
   auto* dV = d.get<tjm::cx<double>>(n * nn);
-  auto* dS = d.get<double>(nn);
+  auto* dS = d.get<double>(nn + 1);      // and the flops
   char* ws = d.get<char>(tjm::svd_call_slots(mm, nn) * 16);
   int* iw = d.get<int>(2 * nn);
   if (!dA || !dU || !dV || !dS || !ws || !iw) return TJM_ENOMEM;
   if (cudaMemcpy(dA, A, (size_t)m * n * 16, cudaMemcpyHostToDevice) != cudaSuccess) return TJM_ECUDA;
   if (double_precision == 2)
     tjm::svd_test_kernel<tjm::df64><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV,
-                                                        reinterpret_cast<tjm::cx<tjm::df64>*>(ws), iw, cut);
+                                                        reinterpret_cast<tjm::cx<tjm::df64>*>(ws), iw, cut, dS + nn);
   else if (double_precision)
     tjm::svd_test_kernel<double><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV, reinterpret_cast<tjm::cx<double>*>(ws), iw,
-                                                 cut);
+                                                 cut, dS + nn);
   else
-    tjm::svd_test_kernel<float><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV, reinterpret_cast<tjm::cx<float>*>(ws), iw, cut);
+    tjm::svd_test_kernel<float><<<1, TJM_THREADS>>>(m, n, dA, dU, dS, dV, reinterpret_cast<tjm::cx<float>*>(ws), iw, cut, dS + nn);
   if (finish()) return TJM_ECUDA;
   cudaMemcpy(U, dU, (size_t)m * nn * 16, cudaMemcpyDeviceToHost);
   cudaMemcpy(V, dV, (size_t)n * nn * 16, cudaMemcpyDeviceToHost);
   cudaMemcpy(S, dS, (size_t)nn * 8, cudaMemcpyDeviceToHost);
+  if (flops) cudaMemcpy(flops, dS + nn, 8, cudaMemcpyDeviceToHost);
   return TJM_OK;
 }
 

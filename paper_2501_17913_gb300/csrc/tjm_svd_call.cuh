@@ -20,10 +20,10 @@ __host__ __device__ constexpr size_t svd_call_slots(int mm, int nn) {
 // A is m x n, row-major complex double; U (m x nn), V (n x nn) row-major, S
 // (nn) descending, A = U diag(S) V^H, nn = min(m, n).  ws holds
 // svd_call_slots(max(m, n), nn) complex T; iw holds 2 nn ints; psm: kSvdSmem bytes of shared memory; cut: see
-// blk_svd_jacobi.  Every workspace entry read is written first, here or inside blk_svd_jacobi.
+// blk_svd_jacobi.  Returns the work in complex multiply-adds.  Every workspace entry read is written first, here or inside blk_svd_jacobi.
 template <class T>
-__device__ void svd_call_body(int m, int n, const cx<double>* A, cx<double>* U, double* S, cx<double>* V, cx<T>* ws,
-                              int* iw, double* red, char* psm, double cut = 0.0) {
+__device__ long long svd_call_body(int m, int n, const cx<double>* A, cx<double>* U, double* S, cx<double>* V, cx<T>* ws,
+                                   int* iw, double* red, char* psm, double cut = 0.0) {
   const bool tr = m < n;
   const int mm = tr ? n : m, nn = tr ? m : n;
   cx<T>* a = ws;
@@ -36,7 +36,8 @@ __device__ void svd_call_body(int m, int n, const cx<double>* A, cx<double>* U, 
     a[e] = tr ? cvt<T>(conj(A[j * n + i])) : cvt<T>(A[i * n + j]);
   }
   __syncthreads();
-  blk_svd_jacobi<T>(mm, nn, a, u, s, v, vw, reinterpret_cast<T*>(vw + nn * nn), iw, red, psm, true, cut);
+  const long long cmacs =
+      blk_svd_jacobi<T>(mm, nn, a, u, s, v, vw, reinterpret_cast<T*>(vw + nn * nn), iw, red, psm, true, cut);
   __syncthreads();
   // the work matrix was A or A^H: return U (m x nn) and V (n x nn) of A
   for (int e = threadIdx.x; e < m * nn; e += TJM_THREADS) {
@@ -48,6 +49,7 @@ __device__ void svd_call_body(int m, int n, const cx<double>* A, cx<double>* U, 
     V[e] = cvt<double>(tr ? u[j * mm + i] : v[j * nn + i]);
   }
   for (int e = threadIdx.x; e < nn; e += TJM_THREADS) S[e] = (double)s[e];
+  return cmacs;
 }
 
 }  // namespace tjm

@@ -109,7 +109,8 @@ SIGNATURES = [
     ("tjm_selftest_svd", C.c_int, [C.c_int, C.c_int, C.c_int, C.POINTER(C.c_double), C.POINTER(C.c_double),
                                    C.POINTER(C.c_double), C.POINTER(C.c_double)]),
     ("tjm_selftest_svd_cut", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_double, C.POINTER(C.c_double),
-                                       C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double)]),
+                                       C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double),
+                                       C.POINTER(C.c_double)]),
     ("tjm_selftest_tc_cgemm", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
                                         C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double)]),
     ("tjm_selftest_contract", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
@@ -410,10 +411,11 @@ def selftest_qr(A, double_precision=True):
     return _z(Q), _z(R)
 
 
-def selftest_svd(A, double_precision=True, cut=0.0):
+def selftest_svd(A, double_precision=True, cut=0.0, flops=None):
     """SVD of one matrix by the kernel's block routine: returns (U, S, V) with A = U diag(S) V^H.
     double_precision: False/0 FP32, True/1 FP64, 2 double-float emulated FP64.  cut: the share of the squared
-    singular values that a truncation of the result may discard (tjm_selftest_svd_cut)."""
+    singular values that a truncation of the result may discard (tjm_selftest_svd_cut).
+    flops: a list that receives the counted real flops."""
     lib = load()
     A = np.asarray(A, dtype=np.complex128)
     m, n = A.shape
@@ -421,10 +423,12 @@ def selftest_svd(A, double_precision=True, cut=0.0):
     a = _cplx(A)
     U = np.zeros((m, nn, 2))
     V = np.zeros((n, nn, 2))
-    S = np.zeros(nn)
-    st = lib.tjm_selftest_svd_cut(int(double_precision), m, n, float(cut), _dp(a), _dp(U), _dp(S), _dp(V))
+    S, fl = np.zeros(nn), np.zeros(1)
+    st = lib.tjm_selftest_svd_cut(int(double_precision), m, n, float(cut), _dp(a), _dp(U), _dp(S), _dp(V), _dp(fl))
     if st != TJM_OK:
         raise TJMError(st, "tjm_selftest_svd_cut")
+    if flops is not None:
+        flops.append(float(fl[0]))
     return _z(U), S, _z(V)
 
 
