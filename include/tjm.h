@@ -361,6 +361,10 @@ tjm_status tjm_selftest_tc_cgemm(int M, int N, int K, int conj_a, int conj_b, in
 tjm_status tjm_selftest_contract(int kind, int precision, int tensor_cores, int chl, int chr, int Dl, int Du, int Dr,
                                  const double* W1, const double* W2, const double* Lenv, const double* Renv,
                                  const double* x, double* y);
+/* The same under a GEMM tile rule of tjm_run_set_tile_rule (0 above). */
+tjm_status tjm_selftest_contract_tiles(int tile_rule, int kind, int precision, int tensor_cores, int chl, int chr,
+                                       int Dl, int Du, int Dr, const double* W1, const double* W2, const double* Lenv,
+                                       const double* Renv, const double* x, double* y);
 
 /* exp(i theta T) e_1 for the k x k (k <= 32) real symmetric tridiagonal
  * T = tridiag(beta, alpha, beta): the Lanczos exponential's small factor

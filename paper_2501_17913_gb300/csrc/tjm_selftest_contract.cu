@@ -21,10 +21,10 @@ template <class Tc, class Td>
 __global__ void __launch_bounds__(TJM_THREADS, 1)
 contract_test_kernel(int kind, SlotDev* S, char* scr, ScratchDims dims, const cx<double>* Lin, int nL, int lb,
                      const cx<double>* Rin, int nR, int rb, const cx<double>* x, int nx, cx<double>* y, int ny,
-                     int chl, int chr, int use_tc) {
+                     int chl, int chr, int use_tc, int tile_rule) {
   extern __shared__ __align__(1024) char smem[];
   tc::cta_setup(&tc_ctl, sizeof(Tc) == 4 && use_tc);
-  if (threadIdx.x == 0) gemm_tile_rule = 0;
+  if (threadIdx.x == 0) gemm_tile_rule = tile_rule;
   __syncthreads();
   Ctx<Tc, Td> c;
   make_ctx(c, S, scr, dims, smem);
@@ -74,7 +74,13 @@ T* upload(DevMem& d, const void* src, size_t bytes) {
 extern "C" tjm_status tjm_selftest_contract(int kind, int precision, int tensor_cores, int chl, int chr, int Dl,
                                             int Du, int Dr, const double* W1, const double* W2, const double* Lenv,
                                             const double* Renv, const double* x, double* y) {
-  if (kind < 0 || kind > 4 || (precision != TJM_PREC_FP64 && precision != TJM_PREC_FP32) || chl < 1 || chr < 1 ||
+  return tjm_selftest_contract_tiles(0, kind, precision, tensor_cores, chl, chr, Dl, Du, Dr, W1, W2, Lenv, Renv, x, y);
+}
+
+extern "C" tjm_status tjm_selftest_contract_tiles(int tile_rule, int kind, int precision, int tensor_cores, int chl,
+                                                  int chr, int Dl, int Du, int Dr, const double* W1, const double* W2,
+                                                  const double* Lenv, const double* Renv, const double* x, double* y) {
+  if (tile_rule < 0 || tile_rule > 1 || kind < 0 || kind > 4 || (precision != TJM_PREC_FP64 && precision != TJM_PREC_FP32) || chl < 1 || chr < 1 ||
       chl > 64 || chr > 64 || Dl < 1 || Dr < 1 || Du < 1 || Dl > 8 || Dr > 8 || Du > 8 || !Lenv || !Renv || !x || !y ||
       (kind != 0 && !W1) || (kind == 2 && !W2))
     return TJM_EINVAL;
@@ -141,13 +147,14 @@ extern "C" tjm_status tjm_selftest_contract(int kind, int precision, int tensor_
     const int sm = tjm::smem_bytes<double, double>(false);
     auto k = tjm::contract_test_kernel<double, double>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    k<<<1, TJM_THREADS, sm>>>(kind, dS, scr, dims, dLin, nL, lb, dRin, nR, rb, dx, nx, dy, ny, chl, chr, 0);
+    k<<<1, TJM_THREADS, sm>>>(kind, dS, scr, dims, dLin, nL, lb, dRin, nR, rb, dx, nx, dy, ny, chl, chr, 0,
+                              tile_rule);
   } else {
     const int sm = tjm::smem_bytes<float, double>(true);
     auto k = tjm::contract_test_kernel<float, double>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     k<<<1, TJM_THREADS, sm>>>(kind, dS, scr, dims, dLin, nL, lb, dRin, nR, rb, dx, nx, dy, ny, chl, chr,
-                              tensor_cores);
+                              tensor_cores, tile_rule);
   }
   e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return TJM_ECUDA;

@@ -116,6 +116,7 @@ SIGNATURES = [
     ("tjm_selftest_contract", C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
                                         C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double),
                                         C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_double)]),
+    ("tjm_selftest_contract_tiles", C.c_int, [C.c_int] * 9 + [C.POINTER(C.c_double)] * 6),
     ("tjm_selftest_expm_tridiag", C.c_int, [C.c_int, C.POINTER(C.c_double), C.POINTER(C.c_double), C.c_double,
                                             C.POINTER(C.c_double)]),
     ("tjm_selftest_philox", C.c_int, [C.c_uint64, C.POINTER(C.c_uint64), C.POINTER(C.c_uint32),
@@ -447,7 +448,7 @@ def selftest_tc_cgemm(A, B, conj_a=False, conj_b=False, a_col_major=False, b_k_c
     return _z(out)
 
 
-def selftest_contract(kind, precision, Lenv, Renv, x, W1=None, W2=None, tensor_cores=True):
+def selftest_contract(kind, precision, Lenv, Renv, x, W1=None, W2=None, tensor_cores=True, tile_rule=0):
     """One effective-Hamiltonian application (kind 0 bond, 1 one site, 2 two sites) or environment update
     (3 left, 4 right) by the trajectory kernel's device functions; layouts as in tjm_selftest_contract."""
     lib = load()
@@ -470,8 +471,9 @@ def selftest_contract(kind, precision, Lenv, Renv, x, W1=None, W2=None, tensor_c
     w2 = _cplx(W2) if W2 is not None else None
     rin = _cplx(Renv) if kind != 3 else np.zeros(2)
     lin = _cplx(Lenv) if kind != 4 else np.zeros(2)
-    st = lib.tjm_selftest_contract(int(kind), int(precision), int(bool(tensor_cores)), int(chl), int(chr_), int(Dl),
-                                   int(Du), int(Dr), _dp(w1), _dp(w2), _dp(lin), _dp(rin), _dp(_cplx(x)), _dp(out))
+    st = lib.tjm_selftest_contract_tiles(int(tile_rule), int(kind), int(precision), int(bool(tensor_cores)), int(chl),
+                                         int(chr_), int(Dl), int(Du), int(Dr), _dp(w1), _dp(w2), _dp(lin), _dp(rin),
+                                         _dp(_cplx(x)), _dp(out))
     if st != TJM_OK:
         raise TJMError(st, "tjm_selftest_contract")
     return _z(out)
