@@ -153,12 +153,6 @@ TJM_HD bool operator>=(df64 a, df64 b) { return !(a < b); }
 TJM_HD bool operator==(df64 a, df64 b) { return a.hi == b.hi && a.lo == b.lo; }
 TJM_HD bool operator!=(df64 a, df64 b) { return !(a == b); }
 
-#if defined(__CUDACC__)
-__device__ __forceinline__ df64 shfl_xor_df(unsigned m, df64 v, int o) {
-  return df64(__shfl_xor_sync(m, v.hi, o), __shfl_xor_sync(m, v.lo, o));
-}
-#endif
-
 }  // namespace tjm
 
 #undef TJM_HD
