@@ -438,14 +438,16 @@ def main():
         t5 = time.perf_counter()
         cpu = oracle_sample(max(1, min(os.cpu_count() or 1, 16)), min(L, a.ref_sites), chi)
         phase_wall["cpu_baseline"] = time.perf_counter() - t5
+    reductions = ("sums across threads: norms and Lanczos coefficients as double-float pairs (2^-48), jump weights, "
+                  "expectation values and truncation sums in FP64")
     if rank == 0:
         out = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps,
                "warmup": a.warmup, "ms_per_step": t_max / a.steps, "higher_is_better": True, "scaling": "weak",
                "vs_baseline": None, "dtype": dtype, "data": "synthetic",
                "arithmetic": {"f32+df64": "FP32 contractions (FP32 accumulation); QR/SVD in double-float emulated "
-                                          "FP64; norms, jump weights, Lanczos coefficients in FP64",
-                              "f32+f64": "FP32 contractions; QR/SVD in native FP64; FP64 reductions",
-                              "f32": "FP32 contractions and QR/SVD; FP64 reductions",
+                                          "FP64; " + reductions,
+                              "f32+f64": "FP32 contractions; QR/SVD in native FP64; " + reductions,
+                              "f32": "FP32 contractions and QR/SVD; " + reductions,
                               "f64": "FP64 throughout"}[a.precision],
                "config": workload_config(a, world, 8 if prec else 16),
                "roofline": roof, "clocks": clocks, "gpu_launches": gpu_launches,

@@ -44,13 +44,15 @@ enum {
 };
 
 /* Arithmetic of the GPU path (the precision plan: contractions in FP32, the
- * QR/SVD truncations, norms, jump probabilities and Lanczos coefficients in
- * FP64).
+ * QR/SVD truncations in FP64 or its emulation; sums across threads that decide
+ * anything in more than FP32: FP64, or double-float pairs of 48 bits).
  *   FP64        everything in double (the plain FP64 baseline).
  *   FP32        tensor contractions and Krylov vectors in complex FP32 with
- *               FP32 accumulation; QR and SVD in native FP64; norms, jump
- *               weights, Lanczos coefficients and expectation values
- *               accumulated in FP64.
+ *               FP32 accumulation; QR and SVD in native FP64; jump weights,
+ *               expectation values, truncation sums and the exponential of
+ *               the Krylov tridiagonal in FP64; norms, jump probabilities
+ *               and Lanczos coefficients summed across threads as
+ *               double-float pairs (2^-48) and rooted in double-float.
  *   FP32_DEC32  as FP32 but QR and SVD in FP32, in shared memory, with
  *               compensated FP32 reductions in the Jacobi SVD and a
  *               Gram-Schmidt pass that keeps the factors orthonormal to FP32
@@ -60,7 +62,10 @@ enum {
  *               significand) on the FP32 pipes.  GB300 executes 2 native FP64
  *               FMAs per clock per SM against 128 FP32 FMAs; the emulation
  *               gives the FP64 factorizations about 3x the native rate with
- *               results equal to native FP64 to ~1e-11 relative. */
+ *               results equal to native FP64 to ~1e-11 relative.
+ * The Jacobi SVD of FP64 and double-float columns finds its first rotations on
+ * an FP32 factor and its later angles from FP32 words, both corrected to unitary
+ * in the factorization's precision, in which it converges. */
 enum { TJM_PREC_FP64 = 0, TJM_PREC_FP32 = 1, TJM_PREC_FP32_DEC32 = 2, TJM_PREC_FP32_DF64 = 3 };
 
 /* Hamiltonian H0 as a matrix product operator (Methods, Sec. "Matrix product

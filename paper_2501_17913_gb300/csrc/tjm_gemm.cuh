@@ -240,8 +240,8 @@ __device__ __noinline__ void gemm_direct(int batch, int M, int N, int K, const c
 // products both are at the unit (bond 64, two CTAs per SM, the later one: 320 x 128 x 64 10.7 M cycles against
 // 10.8 M in whole tiles, 128 x 64 x 320 10.7 / 10.7, 64 x 320 x 128 10.8 / 10.7; least possible 10.5), and with
 // one CTA per SM the direct form waits a little on operands that L1 does not hold (5.67 / 5.44, 5.55 / 5.44, 5.66 / 5.39;
-// least possible 5.24).  Whole FP64 runs at bond 64, one step of L = 16: 1.55 against 1.97 s with one
-// trajectory per SM, 2.77 against 3.57 with two.  So every FP64 product takes it.
+// least possible 5.24).  Whole FP64 runs at bond 64, one step of L = 16: 1.53 against 1.96 s with one
+// trajectory per SM, 2.77 against 3.56 with two.  So every FP64 product takes it.
 constexpr long long kDirectF32 = 8192, kOnePassF32 = 16384;
 
 // Tile choice of the tiled form.  gemm_tile_rule == 0: always 64 x 64 tiles.

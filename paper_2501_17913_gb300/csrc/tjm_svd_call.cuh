@@ -19,8 +19,10 @@ __host__ __device__ constexpr size_t svd_call_slots(int mm, int nn) {
 
 // A is m x n, row-major complex double; U (m x nn), V (n x nn) row-major, S
 // (nn) descending, A = U diag(S) V^H, nn = min(m, n).  ws holds
-// svd_call_slots(max(m, n), nn) complex T; iw holds 2 nn ints; psm: kSvdSmem bytes of shared memory; cut: see
-// blk_svd_jacobi.  Returns the work in complex multiply-adds.  Every workspace entry read is written first, here or inside blk_svd_jacobi.
+// svd_call_slots(max(m, n), nn) complex T; iw holds 2 nn ints; psm: kSvdSmem bytes
+// of shared memory; cut: see blk_svd_jacobi.  Returns the work in complex
+// multiply-adds.  Every workspace entry read is written first, here or inside
+// blk_svd_jacobi.
 template <class T>
 __device__ long long svd_call_body(int m, int n, const cx<double>* A, cx<double>* U, double* S, cx<double>* V, cx<T>* ws,
                                    int* iw, double* red, char* psm, double cut = 0.0) {
