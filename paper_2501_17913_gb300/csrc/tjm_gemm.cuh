@@ -84,11 +84,11 @@ __device__ __forceinline__ void slice_f32(int kn, const cx<float>* As, const cx<
 // slices that are already there (106 to 130 and 70 with whole 64 x 64 tiles, unpadded
 // rows and a bounds check per load).  Copied
 // element by element into two buffers (cp.async) in 128 x 64 tiles: 149 to 163, and 98
-// instead of 138 at 64 x 32 x 160.
+// instead of 138 at 64 x 32 x 160.  Strides between batches are 32-bit like the others (registers are short here).
 template <bool AK, bool BJ, int TM>
 __device__ __noinline__ void gemm_core(int batch, int M, int N, int K, const cx<float>* __restrict__ A, int sai, int sak,
-                                       int ca, long long sa, const cx<float>* __restrict__ B, int sbk, int sbj, int cb,
-                                       long long sb, cx<float>* C, int sci, int scj, long long sc, char* smem) {
+                                       int ca, int sa, const cx<float>* __restrict__ B, int sbk, int sbj, int cb,
+                                       int sb, cx<float>* C, int sci, int scj, int sc, char* smem) {
   constexpr int NQ = TM / 16;              // loads and accumulator rows / columns per thread
   constexpr int KS = TJM_THREADS / TM;     // k rows covered per load round in the i- / j-contiguous layouts
   constexpr int LD = TM + GB_PAD;
@@ -279,11 +279,11 @@ template <bool AK, bool BJ>
 __device__ __forceinline__ void gemm_layout(int batch, int M, int N, int K, MatA<float> A, long long sa, MatB<float> B,
                                             long long sb, cx<float>* C, int sci, int scj, long long sc, char* smem) {
   if (gemm_tile_rule == 1 && (M <= 32 || N <= 32))
-    gemm_core<AK, BJ, 32>(batch, M, N, K, A.p, (int)A.si, (int)A.sk, A.conj, sa, B.p, (int)B.sk, (int)B.sj, B.conj, sb, C,
-                          sci, scj, sc, smem);
+    gemm_core<AK, BJ, 32>(batch, M, N, K, A.p, (int)A.si, (int)A.sk, A.conj, (int)sa, B.p, (int)B.sk, (int)B.sj, B.conj,
+                          (int)sb, C, sci, scj, (int)sc, smem);
   else
-    gemm_core<AK, BJ, 64>(batch, M, N, K, A.p, (int)A.si, (int)A.sk, A.conj, sa, B.p, (int)B.sk, (int)B.sj, B.conj, sb, C,
-                          sci, scj, sc, smem);
+    gemm_core<AK, BJ, 64>(batch, M, N, K, A.p, (int)A.si, (int)A.sk, A.conj, (int)sa, B.p, (int)B.sk, (int)B.sj, B.conj,
+                          (int)sb, C, sci, scj, (int)sc, smem);
 }
 
 // Batched: for b < batch, operands offset by (sa, sb, sc) elements.
