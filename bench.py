@@ -406,10 +406,10 @@ def main():
     if not a.no_fp64 and rank == 0:
         t3 = time.perf_counter()
         ctx3 = tjm.Context(W, jumps, dt, chi, 1e-10, precision=tjm.PREC_FP64, device=local)
-        # FP64 is bound by the SM's FP64 pipe: one CTA per SM already takes nearly all of it (measured at
-        # L = 100: 152 trajectories 669, 304 trajectories 692 trajectory*site*steps/s), while a count between
-        # one and two per SM leaves the two-CTA SMs setting the step time.  One trajectory per SM is the
-        # FP64 path's best use of the GPU per unit of time.
+        # FP64 is bound by the SM's FP64 pipe: one CTA per SM reaches 93 % of the rate of two (measured at
+        # L = 100: 152 trajectories 766, 304 trajectories 823 trajectory*site*steps/s), while a count between
+        # one and two per SM leaves the two-CTA SMs setting the step time.  One trajectory per SM stands for
+        # the path at little more than half the time of a step of two.
         N64 = a.fp64_traj or min(N, n_sm)
         r3 = ctx3.prepare(psi, N64, 0, obs, [dt, 2 * dt])
         ctx3.advance(r3, 0)
